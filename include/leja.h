@@ -272,6 +272,21 @@ ll_status ll_trim_workspace(ll_handle* h);
 enum { LL_INJECT_NONE = 0, LL_INJECT_STALL = 1 };
 ll_status ll_debug_inject(ll_handle* h, int what);
 
+/* Test hook for kernels that LL_KERNEL_AUTO takes by timing and reports as LL_KERNEL_GATHER.
+ *   LL_FAMILY_AUTO     the automatic choice (default);
+ *   LL_FAMILY_STEP     one launch a step, k_leja_step or k_leja_tma only;
+ *   LL_FAMILY_ROWS     k_leja_rows (a row per group of lanes) wherever its layout fits;
+ *   LL_FAMILY_CLUSTER  the cluster-resident pass wherever one fits;
+ *   LL_FAMILY_BAND     reported only: the banded multi-step pass.
+ * From now on the forward, polynomial and backward calls of this handle whose step kernel is automatic
+ * take the family where it applies and choose as under LL_FAMILY_STEP elsewhere (banded passes are
+ * not affected). LL_ERR_INVALID_ARG for another value. */
+enum { LL_FAMILY_AUTO = 0, LL_FAMILY_STEP = 1, LL_FAMILY_ROWS = 2, LL_FAMILY_CLUSTER = 3, LL_FAMILY_BAND = 4 };
+ll_status ll_debug_family(ll_handle* h, int family);
+/* The families that ran: out[0] pass 1 of the last forward (or the last polynomial call), out[1] its
+ * trace pass, out[2] the reverse steps of the last backward (LL_FAMILY_AUTO: none ran). */
+ll_status ll_debug_families_run(const ll_handle* h, int* out);
+
 /* ---- host-side method pieces (FP64 on the host: their stability needs it) ------------------ */
 
 /* First `count` fast Léja points on [-2, 2] into xi_out (host, count doubles).

@@ -30,6 +30,7 @@ LL_STREAM_S, LL_STREAM_G, LL_STREAM_POWER = 0, 1, 2
 LL_KERNEL_AUTO, LL_KERNEL_GATHER, LL_KERNEL_TMA, LL_KERNEL_BAND = 0, 1, 2, 3
 LL_EST_HUTCHPP, LL_EST_HUTCHINSON = 0, 1
 LL_INJECT_NONE, LL_INJECT_STALL = 0, 1
+LL_FAMILY_AUTO, LL_FAMILY_STEP, LL_FAMILY_ROWS, LL_FAMILY_CLUSTER, LL_FAMILY_BAND = 0, 1, 2, 3, 4
 LL_NOALLOC_MAX_ROWS = 1 << 18
 
 
@@ -86,6 +87,8 @@ SIGNATURES = {
     "ll_set_adjoint_fusion": (_I, [_P, _I]),
     "ll_trim_workspace": (_I, [_P]),
     "ll_debug_inject": (_I, [_P, _I]),
+    "ll_debug_family": (_I, [_P, _I]),
+    "ll_debug_families_run": (_I, [_P, ctypes.POINTER(_I)]),
     "ll_leja_points": (_I, [_I, _PD]),
     "ll_divided_differences": (_I, [ll_bounds, _I, _I, _PD, ctypes.POINTER(_I)]),
     "ll_divided_differences_q": (_I, [ll_bounds, _I, _PD]),

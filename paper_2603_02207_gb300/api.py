@@ -17,6 +17,7 @@ from ._ffi import (LL_EST_HUTCHINSON, LL_EST_HUTCHPP, LL_F32, LL_F64, LL_KERNEL_
 
 PRECISIONS = {"f64": LL_PREC_F64, "df64": LL_PREC_DF64, "f32": LL_PREC_F32_MIXED}
 PROBE_KINDS = {"rademacher": LL_PROBE_RADEMACHER, "gaussian": LL_PROBE_GAUSSIAN}
+_FAMILIES = ("auto", "step", "rows", "cluster", "band")   # LL_FAMILY_*
 STEP_KERNELS = {"auto": LL_KERNEL_AUTO, "gather": LL_KERNEL_GATHER, "tma": LL_KERNEL_TMA, "band": LL_KERNEL_BAND}
 ESTIMATORS = {"hutchpp": LL_EST_HUTCHPP, "hutchinson": LL_EST_HUTCHINSON}
 
@@ -86,6 +87,16 @@ class Handle:
     def debug_inject(self, what: str = "none"):
         """Test hook: "stall" makes the TMA step kernel's first-tile waits run out (LL_ERR_TIMEOUT)."""
         self.check(self._lib.ll_debug_inject(self.ptr, {"none": _ffi.LL_INJECT_NONE, "stall": _ffi.LL_INJECT_STALL}[what]))
+
+    def debug_family(self, family: str = "auto"):
+        """Test hook: the kernel family that automatic passes take (auto, step, rows, cluster)."""
+        self.check(self._lib.ll_debug_family(self.ptr, _FAMILIES.index(family)))
+
+    def debug_families_run(self) -> tuple[str, str, str]:
+        """The families of the last pass 1 (or polynomial), trace pass and reverse steps."""
+        out = (ctypes.c_int * 3)()
+        self.check(self._lib.ll_debug_families_run(self.ptr, out))
+        return tuple(_FAMILIES[v] for v in out)
 
     def info(self) -> dict:
         inf = _ffi.ll_info()

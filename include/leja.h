@@ -279,8 +279,8 @@ ll_status ll_debug_inject(ll_handle* h, int what);
  *   LL_FAMILY_CLUSTER  the cluster-resident pass wherever one fits;
  *   LL_FAMILY_BAND     reported only: the banded multi-step pass.
  * From now on the forward, polynomial and backward calls of this handle whose step kernel is automatic
- * take the family where it applies and choose as under LL_FAMILY_STEP elsewhere (banded passes are
- * not affected). LL_ERR_INVALID_ARG for another value. */
+ * take the family where it applies and choose as under LL_FAMILY_STEP elsewhere, on banded
+ * matrices too. LL_ERR_INVALID_ARG for another value. */
 enum { LL_FAMILY_AUTO = 0, LL_FAMILY_STEP = 1, LL_FAMILY_ROWS = 2, LL_FAMILY_CLUSTER = 3, LL_FAMILY_BAND = 4 };
 ll_status ll_debug_family(ll_handle* h, int family);
 /* The families that ran: out[0] pass 1 of the last forward (or the last polynomial call), out[1] its

@@ -220,6 +220,7 @@ cudaError_t rows_typed(const StepLaunch& L, const StepParams& p, bool run, int* 
 }
 
 cudaError_t rows_dispatch(int precision, int mode, int q, const StepLaunch& L, const StepParams& p, bool run, int* per_sm, cudaStream_t s) {
+    if (q < 1 || q > 2) return cudaErrorInvalidValue;
     switch ((precision * NUM_MODES + mode) * 2 + q - 1) {
 #define RUN(P_, M_)                                                                                           \
     case (P_ * NUM_MODES + M_) * 2: return rows_typed<P_, M_, 1>(L, p, run, per_sm, s);                        \

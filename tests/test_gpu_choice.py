@@ -1,0 +1,46 @@
+"""What the cached choice of a step kernel rests on (needs a GB300 and the library)."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from oracle import logdet as O
+from synth import CSR, powerlaw_laplacian
+from tests.gpu_util import lib, need_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    return lib()
+
+
+def _regular(n, nnz):
+    """Rows of nearly equal length with columns next to the diagonal, with n rows and nnz entries."""
+    length = np.full(n, nnz // n)
+    length[: nnz - n * (nnz // n)] += 1
+    rowptr = np.concatenate([[0], np.cumsum(length)]).astype(np.int32)
+    row = np.repeat(np.arange(n), length)
+    start = np.clip(np.arange(n) - length // 2, 0, n - length)
+    col = start[row] + np.arange(nnz) - rowptr[row]
+    return CSR(n, rowptr, col.astype(np.int32), np.where(col == row, 2.0, 0.01))
+
+
+@pytest.mark.parametrize("first", ["irregular", "regular"])
+def test_choice_is_not_taken_over_by_another_kind_of_matrix(L, first):
+    """Two matrices of equal n and nnz on one handle, one of which the row kernel does not suit."""
+    torch = need_gpu()
+    P = powerlaw_laplacian(1 << 17, seed=1)
+    R = _regular(P.n, P.nnz)
+    assert R.nnz == P.nnz
+    V = torch.as_tensor(np.random.default_rng(0).standard_normal((P.n, 40))).cuda()
+    mats = {"irregular": (L.DeviceCSR.from_host(P, "f32"), 0.01, O.gershgorin(P)[1]), "regular": (L.DeviceCSR.from_host(R, "f32"), 1.0, 3.0)}
+    g = L.Handle()
+    g.set_step_config("gather", 0, 0)
+    h = L.Handle()
+    for name in (first, "regular" if first == "irregular" else "irregular"):
+        dA, lo, hi = mats[name]
+        got = L.ll_apply_poly(h, dA, lo, hi, 4, V, "f32")
+        assert h.debug_families_run()[0] == ("rows" if name == "irregular" else "step")
+        assert torch.equal(got, L.ll_apply_poly(g, dA, lo, hi, 4, V, "f32")), name

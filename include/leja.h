@@ -267,9 +267,11 @@ ll_status ll_trim_workspace(ll_handle* h);
  * this handle expects 16 bytes for its first tile that no copy delivers, so that tile's pipeline
  * waits run out after the options' timeout_cycles; the kernel then records the error, stops
  * issuing copies, waits (bounded) for the copies it issued, and returns, and the call fails with
- * LL_ERR_TIMEOUT while the context stays usable. LL_INJECT_NONE clears it. No other kernel is
- * affected. LL_ERR_INVALID_ARG for an unknown value. */
-enum { LL_INJECT_NONE = 0, LL_INJECT_STALL = 1 };
+ * LL_ERR_TIMEOUT while the context stays usable. LL_INJECT_GRAM: from now on, a memset behind each
+ * CholeskyQR2 Gram that this handle launches sets the error flag as a tensor-core Gram whose wait ran out does
+ * (nothing stalls), and the call fails with LL_ERR_TIMEOUT. LL_INJECT_NONE clears both. No other
+ * kernel is affected. LL_ERR_INVALID_ARG for an unknown value. */
+enum { LL_INJECT_NONE = 0, LL_INJECT_STALL = 1, LL_INJECT_GRAM = 2 };
 ll_status ll_debug_inject(ll_handle* h, int what);
 
 /* Test hook for kernels that LL_KERNEL_AUTO takes by timing and reports as LL_KERNEL_GATHER.

@@ -29,7 +29,7 @@ LL_REORDER_AUTO, LL_REORDER_NONE, LL_REORDER_DEGREE = 0, 1, 2
 LL_STREAM_S, LL_STREAM_G, LL_STREAM_POWER = 0, 1, 2
 LL_KERNEL_AUTO, LL_KERNEL_GATHER, LL_KERNEL_TMA, LL_KERNEL_BAND = 0, 1, 2, 3
 LL_EST_HUTCHPP, LL_EST_HUTCHINSON = 0, 1
-LL_INJECT_NONE, LL_INJECT_STALL = 0, 1
+LL_INJECT_NONE, LL_INJECT_STALL, LL_INJECT_GRAM = 0, 1, 2
 LL_FAMILY_AUTO, LL_FAMILY_STEP, LL_FAMILY_ROWS, LL_FAMILY_CLUSTER, LL_FAMILY_BAND = 0, 1, 2, 3, 4
 LL_NOALLOC_MAX_ROWS = 1 << 18
 

@@ -86,7 +86,8 @@ class Handle:
 
     def debug_inject(self, what: str = "none"):
         """Test hook: "stall" makes the TMA step kernel's first-tile waits run out (LL_ERR_TIMEOUT)."""
-        self.check(self._lib.ll_debug_inject(self.ptr, {"none": _ffi.LL_INJECT_NONE, "stall": _ffi.LL_INJECT_STALL}[what]))
+        self.check(self._lib.ll_debug_inject(self.ptr, {"none": _ffi.LL_INJECT_NONE, "stall": _ffi.LL_INJECT_STALL,
+                                                         "gram": _ffi.LL_INJECT_GRAM}[what]))
 
     def debug_family(self, family: str = "auto"):
         """Test hook: the kernel family that automatic passes take (auto, step, rows, cluster)."""

@@ -3,25 +3,26 @@
 // the sparsity pattern), the initial Lambda_m = d_m U, the row index of every stored entry, and the
 // chain to model parameters sum_e g_e da_e/dtheta_p.
 #include "common.cuh"
+#include "index_range.h"
 #include "kernels.cuh"
 #include "step_common.cuh"
 
 namespace ll {
 
 __global__ void k_row_index(const int32_t* rowptr, int n, int32_t* rowidx) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i = step_to(i, (int)(gridDim.x * blockDim.x), n))
         for (int e = rowptr[i]; e < rowptr[i + 1]; ++e) rowidx[e] = i;
 }
 
 // tmap[e] = the index of entry (c, r) for every stored entry e = (r, c) of a pattern whose rows hold
 // strictly increasing columns (binary search in row c); flag[0] |= 1 where (c, r) is not stored
 __global__ void k_transpose_map(const int32_t* rowptr, const int32_t* colind, int n, int32_t* tmap, int* flag) {
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
+    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r = step_to(r, (int)(gridDim.x * blockDim.x), n)) {
         for (int e = rowptr[r]; e < rowptr[r + 1]; ++e) {
             const int c = colind[e];
             int lo = rowptr[c], hi = rowptr[c + 1];
             while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
+                const int mid = lo + ((hi - lo) >> 1);
                 if (colind[mid] < r) lo = mid + 1; else hi = mid;
             }
             if (lo < rowptr[c + 1] && colind[lo] == r) {

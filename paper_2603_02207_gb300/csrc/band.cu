@@ -13,6 +13,7 @@
 // diagonals are visited in ascending column order (the CSR order), so P and W match the
 // one-step kernels bit for bit. The traces are summed over rows in another order.
 #include "common.cuh"
+#include "index_range.h"
 #include "kernels.cuh"
 #include "step_common.cuh"
 
@@ -217,7 +218,7 @@ __global__ void __launch_bounds__(BAND_THREADS) k_leja_band(const BandParams bp)
 // have been checked to hold strictly increasing columns within two of the diagonal.
 template <typename Raw>
 __global__ void k_to_dia(const int32_t* rowptr, const int32_t* colind, const Raw* vals, int n, Raw* dia) {
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
+    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r = step_to(r, (int)(gridDim.x * blockDim.x), n)) {
         Raw v[BAND_D];
 #pragma unroll
         for (int d = 0; d < BAND_D; ++d) v[d] = Raw{};

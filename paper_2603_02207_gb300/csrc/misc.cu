@@ -4,6 +4,7 @@
 
 #include "common.cuh"
 #include "gauss.cuh"
+#include "index_range.h"
 #include "kernels.cuh"
 
 namespace ll {
@@ -37,7 +38,7 @@ __global__ void k_probes(int kind, uint64_t seed, int stream_id, int n, int cols
     const int col0 = (int)threadIdx.x - roff * (narrow ? pad : 0);
     const int cstep = narrow ? pad : nt;
     if (roff >= rpb) return;
-    for (int row = blockIdx.x * rpb + roff; row < n; row += gridDim.x * rpb) {
+    for (int row = blockIdx.x * rpb + roff; row < n; row = step_to(row, (int)(gridDim.x * rpb), n)) {
         const uint32_t prow = (uint32_t)(rowmap ? rowmap[row] : row);   // the row whose probe values these are
         for (int col = col0; col < pad; col += cstep) {
             const size_t idx = (size_t)row * ld + col;
@@ -84,7 +85,7 @@ __device__ __forceinline__ bool csr_has(const int32_t* rowptr, const int32_t* co
     int lo = rowptr[i], hi = rowptr[i + 1];
     if (lo < 0 || hi < lo || (int64_t)hi > nnz) return false;
     while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
+        const int mid = lo + ((hi - lo) >> 1);
         if (colind[mid] < c) lo = mid + 1; else hi = mid;
     }
     return lo < rowptr[i + 1] && colind[lo] == c;
@@ -143,7 +144,7 @@ __global__ void __launch_bounds__(256) k_validate_csr(const int32_t* rowptr, con
             const int a = rowptr[i], e = rowptr[i + 1];
             bool inc = true;
 #pragma unroll 4
-            for (int k = a + lane; k < e; k += 32) {
+            for (int k = step_to(a, lane, e); k < e; k = step_to(k, 32, e)) {
                 const int c = colind[k];
                 const int prev = k > a ? colind[k - 1] : -1;
                 if (c < 0 || c >= n) atomicOr(flag, 2);
@@ -179,17 +180,17 @@ cudaError_t launch_validate_csr(const int32_t* rowptr, const int32_t* colind, in
 template <typename T>
 __global__ void k_check_symmetric(const int32_t* rowptr, const int32_t* colind, const T* vals, int n, int sorted,
                                   int* flag) {
-    for (int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < n; r += gridDim.x * (blockDim.x >> 5)) {
+    for (int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < n; r = step_to(r, (int)(gridDim.x * (blockDim.x >> 5)), n)) {
         const int k0 = rowptr[r], k1 = rowptr[r + 1];
         bool bad = false;
-        for (int k = k0 + (threadIdx.x & 31); k < k1; k += 32) {
+        for (int k = step_to(k0, threadIdx.x & 31, k1); k < k1; k = step_to(k, 32, k1)) {
             const int c = colind[k];
             const T v = vals[k];
             int lo = rowptr[c], hi = rowptr[c + 1];
             bool found = false;
             if (sorted) {
                 while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
+                    const int mid = lo + ((hi - lo) >> 1);
                     const int cm = colind[mid];
                     if (cm == r) { found = vals[mid] == v; break; }
                     if (cm < r) lo = mid + 1; else hi = mid;
@@ -218,7 +219,7 @@ template <typename T>
 __global__ void k_gershgorin(const int32_t* rowptr, const int32_t* colind, const T* vals, int n,
                              double* partials, unsigned int* ticket, double* out) {
     double lo = INFINITY, hi = -INFINITY;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i = step_to(i, (int)(gridDim.x * blockDim.x), n)) {
         double a_ii = 0.0, r_i = 0.0;
         for (int k = rowptr[i]; k < rowptr[i + 1]; ++k) {
             const double v = (double)vals[k];
@@ -329,7 +330,7 @@ cudaError_t launch_prepare_values(const void* vals, int dtype, int64_t nnz, doub
 template <typename TI, typename TO>
 __global__ void k_prepare_pencil(const int32_t* rowptr, const int32_t* colind, const TI* o, const double* D, int n,
                                  double theta, double scale, TO* out, int* flag) {
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
+    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r = step_to(r, (int)(gridDim.x * blockDim.x), n)) {
         const double dr = D[r];
         int nd = 0;
         for (int e = rowptr[r]; e < rowptr[r + 1]; ++e) {
@@ -483,7 +484,7 @@ cudaError_t launch_scaled_copy_f64(const double* in, long long ld_in, double* ou
 
 template <typename T>
 __global__ void k_unit_diag(T* out, long long ld, int n) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i = step_to(i, (int)(gridDim.x * blockDim.x), n))
         store_f64<T>(out, (size_t)i * ld + i, 1.0);
 }
 
@@ -500,7 +501,7 @@ cudaError_t launch_unit_diag(int t, void* out, long long ld, int n, cudaStream_t
 // ----------------------------------------------------------------- power iteration (FP64)
 template <typename T>
 __global__ void k_spmv(const int32_t* rowptr, const int32_t* colind, const T* vals, int n, const double* x, double* y) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i = step_to(i, (int)(gridDim.x * blockDim.x), n)) {
         double acc = 0.0;
         for (int k = rowptr[i]; k < rowptr[i + 1]; ++k) acc = fma((double)vals[k], x[colind[k]], acc);
         y[i] = acc;
@@ -516,7 +517,7 @@ cudaError_t launch_spmv_f64(const int32_t* rowptr, const int32_t* colind, const 
 
 __global__ void k_dot(const double* x, const double* y, int n, double* partials, unsigned int* ticket, double* out) {
     double acc = 0.0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) acc = fma(x[i], y[i], acc);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i = step_to(i, (int)(gridDim.x * blockDim.x), n)) acc = fma(x[i], y[i], acc);
     __shared__ double s[256];
     __shared__ bool s_last;
     s[threadIdx.x] = acc;
@@ -620,7 +621,7 @@ cudaError_t launch_stop_init(int precision, const void* W0, long long ld, int n,
 // mode 0: x /= sqrt(*num)
 __global__ void k_scale(double* x, const double* num, int n, int mode) {
     const double f = 1.0 / sqrt(*num);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) x[i] *= f;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i = step_to(i, (int)(gridDim.x * blockDim.x), n)) x[i] *= f;
 }
 
 cudaError_t launch_scale_f64(double* x, const double* num, int n, int mode, cudaStream_t s) {

@@ -16,6 +16,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "index_range.h"
 #include "kernels.cuh"
 
 namespace ll {
@@ -36,8 +37,8 @@ __global__ void k_order_hist(const int32_t* rowptr, int n, int* counts) {
     __shared__ int h[ORD_BUCKETS];
     for (int b = threadIdx.x; b < ORD_BUCKETS; b += blockDim.x) h[b] = 0;
     __syncthreads();
-    const int r0 = blockIdx.x * ORD_CHUNK, r1 = min(n, r0 + ORD_CHUNK);
-    for (int r = r0 + (int)threadIdx.x; r < r1; r += blockDim.x) atomicAdd(&h[row_bucket(rowptr, r)], 1);
+    const int r0 = blockIdx.x * ORD_CHUNK, r1 = step_to(r0, ORD_CHUNK, n);
+    for (int r = step_to(r0, (int)threadIdx.x, r1); r < r1; r = step_to(r, (int)blockDim.x, r1)) atomicAdd(&h[row_bucket(rowptr, r)], 1);
     __syncthreads();
     for (int b = threadIdx.x; b < ORD_BUCKETS; b += blockDim.x) counts[(size_t)blockIdx.x * ORD_BUCKETS + b] = h[b];
 }
@@ -79,9 +80,9 @@ __global__ void k_order_scatter(const int32_t* rowptr, int n, const int* offsets
     if (threadIdx.x >= 32) return;
     const int lane = threadIdx.x;
     const unsigned lt = (1u << lane) - 1u;
-    const int r0 = blockIdx.x * ORD_CHUNK, r1 = min(n, r0 + ORD_CHUNK);
-    for (int g = r0; g < r1; g += 32) {
-        const int r = g + lane;
+    const int r0 = blockIdx.x * ORD_CHUNK, r1 = step_to(r0, ORD_CHUNK, n);
+    for (int g = r0; g < r1; g = step_to(g, 32, r1)) {
+        const int r = step_to(g, lane, r1);
         const bool ok = r < r1;
         const int b = ok ? row_bucket(rowptr, r) : -1 - lane;   // distinct keys for the idle lanes
         const unsigned m = __match_any_sync(0xffffffffu, b);
@@ -99,7 +100,7 @@ __global__ void k_order_scatter(const int32_t* rowptr, int n, const int* offsets
 
 // newdeg[i] = entries of old row perm[i]
 __global__ void k_perm_degrees(const int32_t* rowptr, const int32_t* perm, int n, int* newdeg) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i = step_to(i, (int)(gridDim.x * blockDim.x), n)) {
         const int o = perm[i];
         newdeg[i] = rowptr[o + 1] - rowptr[o];
     }
@@ -112,7 +113,7 @@ __global__ void k_scan_blocks(const int* x, int n, int* bsum) {
     __shared__ int s[ORD_THREADS];
     const int b0 = blockIdx.x * ORD_SCAN;
     int t = 0;
-    for (int i = threadIdx.x; i < ORD_SCAN && b0 + i < n; i += blockDim.x) t += x[b0 + i];
+    for (int i = threadIdx.x; i < ORD_SCAN && i < n - b0; i += blockDim.x) t += x[b0 + i];
     s[threadIdx.x] = t;
     __syncthreads();
     for (int w = blockDim.x / 2; w > 0; w >>= 1) {
@@ -135,7 +136,7 @@ __global__ void k_scan_sums(int* bsum, int nb, int* total) {
 __global__ void k_scan_apply(const int* x, int n, const int* boff, int32_t* out) {
     __shared__ int s[ORD_SCAN];
     const int b0 = blockIdx.x * ORD_SCAN;
-    for (int i = threadIdx.x; i < ORD_SCAN; i += blockDim.x) s[i] = b0 + i < n ? x[b0 + i] : 0;
+    for (int i = threadIdx.x; i < ORD_SCAN; i += blockDim.x) s[i] = i < n - b0 ? x[b0 + i] : 0;
     __syncthreads();
     if (threadIdx.x == 0) {
         int acc = boff[blockIdx.x];
@@ -146,7 +147,7 @@ __global__ void k_scan_apply(const int* x, int n, const int* boff, int32_t* out)
         }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < ORD_SCAN && b0 + i < n; i += blockDim.x) out[b0 + i] = s[i];
+    for (int i = threadIdx.x; i < ORD_SCAN && i < n - b0; i += blockDim.x) out[b0 + i] = s[i];
 }
 
 // one warp per new row: its entries copied from the old row with the columns relabelled
@@ -154,10 +155,10 @@ __global__ void k_permute_csr(const int32_t* rowptr, const int32_t* colind, int 
                               const int32_t* inv, const int32_t* rowptr_new, int32_t* colind_new, int32_t* src) {
     const int lane = threadIdx.x & 31;
     const int wpb = blockDim.x >> 5;
-    for (int i = blockIdx.x * wpb + (threadIdx.x >> 5); i < n; i += gridDim.x * wpb) {
+    for (int i = blockIdx.x * wpb + (threadIdx.x >> 5); i < n; i = step_to(i, (int)(gridDim.x * wpb), n)) {
         const int o = perm[i];
         const int a = rowptr[o], e = rowptr[o + 1], d = rowptr_new[i];
-        for (int k = a + lane; k < e; k += 32) {
+        for (int k = step_to(a, lane, e); k < e; k = step_to(k, 32, e)) {
             colind_new[d + (k - a)] = inv[colind[k]];
             src[d + (k - a)] = k;
         }
@@ -195,8 +196,8 @@ size_t reorder_work_bytes(int n) {
 cudaError_t launch_reorder(const int32_t* rowptr, const int32_t* colind, int n, int32_t* perm, int32_t* inv,
                            int32_t* rowptr_new, int32_t* colind_new, int32_t* src, void* work, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    const int nchunks = (n + ORD_CHUNK - 1) / ORD_CHUNK;
-    const int nb = (n + ORD_SCAN - 1) / ORD_SCAN;
+    const int nchunks = (int)(((size_t)n + ORD_CHUNK - 1) / ORD_CHUNK);
+    const int nb = (int)(((size_t)n + ORD_SCAN - 1) / ORD_SCAN);
     int* counts = static_cast<int*>(work);
     int* offsets = counts + (size_t)nchunks * ORD_BUCKETS;
     int* newdeg = offsets + (size_t)nchunks * ORD_BUCKETS;
@@ -205,14 +206,14 @@ cudaError_t launch_reorder(const int32_t* rowptr, const int32_t* colind, int n, 
     k_order_hist<<<nchunks, ORD_THREADS, 0, s>>>(rowptr, n, counts);
     k_order_offsets<<<1, 1024, 0, s>>>(counts, nchunks, offsets);
     k_order_scatter<<<nchunks, 256, 0, s>>>(rowptr, n, offsets, perm, inv);
-    const int g = std::min(152 * 16, (n + ORD_THREADS - 1) / ORD_THREADS);
+    const int g = (int)std::min<size_t>(152 * 16, ((size_t)n + ORD_THREADS - 1) / ORD_THREADS);
     k_perm_degrees<<<g, ORD_THREADS, 0, s>>>(rowptr, perm, n, newdeg);
     k_scan_blocks<<<nb, ORD_THREADS, 0, s>>>(newdeg, n, bsum);
     k_scan_sums<<<1, 32, 0, s>>>(bsum, nb, total);
     k_scan_apply<<<nb, ORD_THREADS, 0, s>>>(newdeg, n, bsum, rowptr_new);
     cudaError_t e = cudaMemcpyAsync(rowptr_new + n, total, sizeof(int), cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess) return e;
-    k_permute_csr<<<std::min(152 * 16, (n + 7) / 8), 256, 0, s>>>(rowptr, colind, n, perm, inv, rowptr_new, colind_new, src);
+    k_permute_csr<<<(int)std::min<size_t>(152 * 16, ((size_t)n + 7) / 8), 256, 0, s>>>(rowptr, colind, n, perm, inv, rowptr_new, colind_new, src);
     return cudaGetLastError();
 }
 

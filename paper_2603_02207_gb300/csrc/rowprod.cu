@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(RP_MAX_WARPS * 32, 2) k_rows_df(const RowProdP
     const int xrow = (int)q.ldx * 8, grow = q.G ? q.kg * 8 : 0;
     const int xbytes = q.TR * xrow, gbytes = (q.TR * grow + 15) & ~15;
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
-    const int ntiles = (q.n + q.TR - 1) / q.TR;
+    const int ntiles = (int)(((long long)q.n + q.TR - 1) / q.TR);
 
     auto stage = [&](int tile, int buf) {
         if (tile < ntiles) {
@@ -256,7 +256,7 @@ cudaError_t rows_df_launch(RowProdParams q, cudaStream_t s) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rows_df, warps * 32, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidValue;
-    const int ntiles = (q.n + q.TR - 1) / q.TR;
+    const int ntiles = (int)(((long long)q.n + q.TR - 1) / q.TR);
     k_rows_df<<<std::min(ntiles, per_sm * 152), warps * 32, smem, s>>>(q);
     return cudaGetLastError();
 }

@@ -21,6 +21,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "index_range.h"
 #include "kernels.cuh"
 #include "step_common.cuh"
 
@@ -44,16 +45,6 @@ __device__ __forceinline__ T ld_once(const T* p) {
 template <typename T>
 __device__ __forceinline__ void st_once(T* p, const T& v) {
     __stcs(reinterpret_cast<float4*>(p), *reinterpret_cast<const float4*>(&v));
-}
-
-// first i in [0, n] with rowptr[i] + ROW_COST i >= t
-__device__ __forceinline__ int rows_start(const int* rowptr, int n, long long t) {
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if ((long long)rowptr[mid] + (long long)ROW_COST * mid >= t) hi = mid; else lo = mid + 1;
-    }
-    return lo;
 }
 
 template <int PREC, int MODE, int Q>
@@ -102,11 +93,11 @@ __global__ void __launch_bounds__(ROWS_THREADS, 2) k_leja_rows(const StepParams 
     const long long w = (long long)blockIdx.x * (ROWS_THREADS / 32) + warp;
     // (the quotient taken first keeps the products in range)
     const long long quo = total / nw, rem = total - quo * nw;
-    const int r0 = rows_start(rowptr, n, w * quo + min(w, rem));
-    const int r1 = w + 1 == nw ? n : rows_start(rowptr, n, (w + 1) * quo + min(w + 1, rem));
+    const int r0 = rows_start(rowptr, n, ROW_COST, w * quo + min(w, rem));
+    const int r1 = w + 1 == nw ? n : rows_start(rowptr, n, ROW_COST, (w + 1) * quo + min(w + 1, rem));
 
     // (the bounds of the next row and of the one after it are there before they are needed)
-    int r = r0 + grp;
+    int r = step_to(r0, grp, r1);
     auto bounds = [&](int row, int& a, int& b) {
         a = b = 0;
         if (on && row < r1) {
@@ -116,10 +107,10 @@ __global__ void __launch_bounds__(ROWS_THREADS, 2) k_leja_rows(const StepParams 
     };
     int k0, k1, m0, m1;
     bounds(r, k0, k1);
-    bounds(r + groups, m0, m1);
+    bounds(step_to(r, groups, r1), m0, m1);
     while (on && r < r1) {
         int z0, z1;
-        bounds(r + 2 * groups, z0, z1);
+        bounds(step_to(r, 2 * groups, r1), z0, z1);
         X wr[Q] = {}, vr[Q] = {}, v2r[Q] = {};
         PP po[NP] = {}, pn[NP];
         load(wr, win + (size_t)r * ldq);
@@ -139,10 +130,11 @@ __global__ void __launch_bounds__(ROWS_THREADS, 2) k_leja_rows(const StepParams 
             if (p.v2) load(v2r, static_cast<const WP*>(p.v2) + (size_t)r * ldq);
         }
         RowAcc A[NP];
-        for (int k = k0; k < k1; k += U) {
+        for (int k = k0; k < k1; k = step_to(k, U, k1)) {
             X x[U][Q];
             Raw av[U];
-            const bool full = k + U <= k1;
+            const int left = k1 - k;
+            const bool full = left >= U;
             if (full) {
 #pragma unroll
                 for (int u = 0; u < U; ++u) av[u] = __ldg(vals + k + u);
@@ -151,13 +143,13 @@ __global__ void __launch_bounds__(ROWS_THREADS, 2) k_leja_rows(const StepParams 
             } else {
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    if (k + u < k1) {
+                    if (u < left) {
                         av[u] = __ldg(vals + k + u);
                         load(x[u], win + (size_t)__ldg(colind + k + u) * ldq);
                     }
                 }
             }
-            const int pf = min(k + ROWS_AHEAD, nnz - 1);
+            const int pf = step_to(k, ROWS_AHEAD, nnz - 1);
             asm volatile("prefetch.global.L1 [%0];" ::"l"(colind + pf));
             asm volatile("prefetch.global.L1 [%0];" ::"l"(vals + pf));
             if (full) {
@@ -170,7 +162,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, 2) k_leja_rows(const StepParams 
             } else {
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    if (k + u < k1) {
+                    if (u < left) {
                         const auto ex = expand(av[u]);
 #pragma unroll
                         for (int y = 0; y < NP; ++y) row_mac<PREC>(A[y], ex, x[u][y / PU].w[y % PU]);
@@ -197,7 +189,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, 2) k_leja_rows(const StepParams 
             for (int y = 0; y < NP; ++y)
                 if (has[y / PU]) st_once(pblk + (size_t)r * ldpq + cp0 + y, pn[y]);
         }
-        r += groups;
+        r = step_to(r, groups, r1);
         k0 = m0;
         k1 = m1;
         m0 = z0;
@@ -274,7 +266,7 @@ bool plan_step_rows(int precision, int mode, int n, int b, StepParams& p, StepLa
         cudaGetLastError();
         return false;
     }
-    L.grid = std::max(1, std::min(per_sm * sm_count, (n + p.rl - 1) / p.rl));
+    L.grid = (int)std::min<long long>((long long)per_sm * sm_count, ((long long)n + p.rl - 1) / p.rl);
     return true;
 }
 

@@ -319,6 +319,12 @@ ll_status ll_divided_differences(ll_bounds bounds, int degree, int sval_mode, do
  * lmin >= lmax, non-finite), LL_ERR_UNSUPPORTED (degree > 100000). */
 ll_status ll_divided_differences_q(ll_bounds bounds, int degree, double* d_out);
 
+/* c_0 .. c_degree of the polynomial sum_j d_j prod_{k<j} (x - xi_k) over the Léja points in the basis
+ * 1, D_1, D_2, ... with D_k(2 cos t) = 2 cos kt, in which the forwards' trace passes sum their moments
+ * (double-double arithmetic, rounded to FP64). d, c_out: host, degree+1 doubles. Errors:
+ * LL_ERR_INVALID_ARG, LL_ERR_UNSUPPORTED (degree > 100000). */
+ll_status ll_moment_coefficients(int degree, const double* d, double* c_out);
+
 /* ---- device kernels exposed for parity checks ---------------------------------------------- */
 
 /* Gershgorin interval [min_i (a_ii - R_i), max_i (a_ii + R_i)], R_i = sum_{j!=i} |a_ij|

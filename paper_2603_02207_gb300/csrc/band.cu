@@ -28,14 +28,15 @@ __host__ __device__ inline size_t a16(size_t x) { return (x + 15) & ~(size_t)15;
 // Shared-memory layout for R rows and tp column pairs (element sizes of the precision)
 struct BandSmem {
     size_t w0, w1, dia, aux, bytes;
-    __host__ __device__ BandSmem(int R, int tp, size_t wpair, size_t raw, size_t auxpair) {
+    // mom: aux holds E of every row of the buffers
+    __host__ __device__ BandSmem(int R, int tp, size_t wpair, size_t raw, size_t auxpair, bool mom) {
         const size_t rb = (size_t)R + 2 * BAND_SMAX * BAND_H;
         const size_t rd = (size_t)R + 2 * (BAND_SMAX - 1) * BAND_H;
         w0 = 0;
         w1 = a16(rb * tp * wpair);
         dia = w1 + a16(rb * tp * wpair);
         aux = dia + a16(rd * BAND_D * raw);
-        bytes = aux + a16((size_t)R * tp * auxpair);
+        bytes = aux + a16((mom ? rb : (size_t)R) * tp * auxpair);
     }
 };
 
@@ -47,13 +48,13 @@ __global__ void __launch_bounds__(BAND_THREADS) k_leja_band(const BandParams bp)
     extern __shared__ __align__(16) unsigned char smem[];
     const int tid = threadIdx.x;
     const int tp = bp.tp, R = bp.R, s = bp.s, n = bp.n;
-    constexpr bool MOM = mom_mode(MODE);   // (see MODE_MOMENT: W_{j-1} starts in the second buffer)
+    constexpr bool MOM = mom_mode(MODE);   // (see MODE_MOMENT)
     constexpr bool DOT = base_mode(MODE) == MODE_DOT;
-    const BandSmem L(R, tp, sizeof(WP), sizeof(Raw), MOM ? 0 : (MODE == MODE_ACCUM ? sizeof(PP) : sizeof(WP)));
+    const BandSmem L(R, tp, sizeof(WP), sizeof(Raw), MODE == MODE_ACCUM ? sizeof(PP) : sizeof(WP), MOM);
     WP* const wbuf0 = reinterpret_cast<WP*>(smem + L.w0);
     WP* const wbuf1 = reinterpret_cast<WP*>(smem + L.w1);
     Raw* const ds = reinterpret_cast<Raw*>(smem + L.dia);
-    WP* const vs = reinterpret_cast<WP*>(smem + L.aux);    // pass 2: the tile's V rows
+    WP* const vs = reinterpret_cast<WP*>(smem + L.aux);    // pass 2: the tile's V rows; moments: E_{j-1}, then E_j
     PP* const ps = reinterpret_cast<PP*>(smem + L.aux);    // pass 1: the tile's P rows
     const int rl = tid / tp, cp = tid - rl * tp;
     const int RL = BAND_THREADS / tp;
@@ -63,8 +64,8 @@ __global__ void __launch_bounds__(BAND_THREADS) k_leja_band(const BandParams bp)
     WP* __restrict__ wout = static_cast<WP*>(bp.wout);
     const Raw* __restrict__ dia = static_cast<const Raw*>(bp.dia);
     const WP* __restrict__ vg = static_cast<const WP*>(bp.v);
-    const WP* __restrict__ wprev = static_cast<const WP*>(bp.wprev);
-    WP* __restrict__ wout2 = static_cast<WP*>(bp.wout2);
+    const WP* __restrict__ ein = static_cast<const WP*>(bp.ein);
+    WP* __restrict__ eout = static_cast<WP*>(bp.eout);
     PP* __restrict__ pg = static_cast<PP*>(bp.p);
     const int hs = s * BAND_H;   // input halo of this launch
 
@@ -78,7 +79,7 @@ __global__ void __launch_bounds__(BAND_THREADS) k_leja_band(const BandParams bp)
             const int row = wbase + rr;
             wbuf0[idx] = (row >= 0 && row < n) ? win[(size_t)row * ldq + c] : WP{};
             if constexpr (MOM) {
-                if (bp.j0 > 0) wbuf1[idx] = (row >= 0 && row < n) ? wprev[(size_t)row * ldq + c] : WP{};
+                if (bp.j0 > 0) vs[idx] = (row >= 0 && row < n) ? ein[(size_t)row * ldq + c] : WP{};
             }
         }
         const int dbase = r0 - (s - 1) * BAND_H;      // row of diagonal index 0
@@ -108,7 +109,7 @@ __global__ void __launch_bounds__(BAND_THREADS) k_leja_band(const BandParams bp)
                 p.beta_df = bp.beta_df[q];
                 p.d0_df = bp.d0_df;
                 p.dn_df = bp.dn_df[q];
-                p.mcoef = bp.j0 + q == 1 ? -2.f : -1.f;
+                p.mcoef = p.first ? -2.f : -1.f;
                 const StepScalars<PREC> S(p, cp);
                 // rows computed at this step: the tile and a halo of (s - 1 - q) * BAND_H rows
                 const int lo = r0 - (s - 1 - q) * BAND_H, hi = r0 + R + (s - 1 - q) * BAND_H;
@@ -126,13 +127,14 @@ __global__ void __launch_bounds__(BAND_THREADS) k_leja_band(const BandParams bp)
                         const WP wr = bin[(size_t)bi * tp + cp];
                         WP* wo = bout + (size_t)bi * tp + cp;
                         if constexpr (MOM) {
-                            // W_{j-1}'s row gives way to W_{j+1}'s; halo rows leave no traces
-                            const WP prev = *wo;
+                            // E_{j-1}'s row gives way to E_j's; halo rows leave no traces
+                            WP* eo = vs + (size_t)bi * tp + cp;
+                            const WP prev = *eo;
                             if (row >= r0 && row < r0 + R && row < n) {
-                                row_epilogue<PREC, MODE>(p, S, A, wr, prev, PP{}, wo, nullptr, T[q]);
+                                row_epilogue<PREC, MODE>(p, S, A, wr, prev, PP{}, wo, nullptr, T[q], WP{}, eo);
                             } else {
                                 TracePart halo;
-                                row_epilogue<PREC, MODE>(p, S, A, wr, prev, PP{}, wo, nullptr, halo);
+                                row_epilogue<PREC, MODE>(p, S, A, wr, prev, PP{}, wo, nullptr, halo, WP{}, eo);
                             }
                         } else if (row >= r0 && row < r0 + R && row < n) {
                             const int ti = (row - r0) * tp + cp;
@@ -151,14 +153,14 @@ __global__ void __launch_bounds__(BAND_THREADS) k_leja_band(const BandParams bp)
                 bout = t;
             }
         }
-        // W_{j+s} (in bin now) and P of the tile's rows; moments: W_{j+s-1} too, and nothing after the last
+        // W_{j+s} (in bin now) and P of the tile's rows; moments: E_{j+s-1} too, and nothing after the last
         for (int idx = tid; idx < R * tp; idx += BAND_THREADS) {
             const int rr = idx / tp, c = idx - rr * tp;
             const int row = r0 + rr;
             if (row < n) {
                 if (!MOM || wout) wout[(size_t)row * ldq + c] = bin[(size_t)(row - wbase) * tp + c];
                 if constexpr (MOM) {
-                    if (wout2) wout2[(size_t)row * ldq + c] = bout[(size_t)(row - wbase) * tp + c];
+                    if (eout) eout[(size_t)row * ldq + c] = vs[(size_t)(row - wbase) * tp + c];
                 }
                 if constexpr (MODE == MODE_ACCUM) pg[(size_t)row * ldpq + c] = ps[idx];
             }
@@ -259,13 +261,16 @@ bool plan_band(int precision, int mode, int n, int b, int sm_count, BandLaunch& 
     if (tp > BAND_THREADS) return false;
     const size_t wpair = precision == LL_PREC_F32_MIXED ? 8 : 16;
     const size_t raw = precision == LL_PREC_F32_MIXED ? 4 : 8;
-    const size_t auxpair = mom_mode(mode) ? 0 : (mode == MODE_ACCUM ? 16 : wpair);
+    const size_t auxpair = mode == MODE_ACCUM ? 16 : wpair;
+    const bool mom = mom_mode(mode);
     // the most rows per tile (a multiple of 32, at most 512) within 72 KB of shared memory, so that
     // three CTAs share an SM and one loads while the others compute
     int R = 512;
-    while (R > 32 && BandSmem(R, tp, wpair, raw, auxpair).bytes > 72 * 1024) R -= 32;
+    while (R > 32 && BandSmem(R, tp, wpair, raw, auxpair, mom).bytes > 72 * 1024) R -= 32;
+    // (the widest moment passes, with three buffers)
+    if (BandSmem(R, tp, wpair, raw, auxpair, mom).bytes > 200 * 1024) R = 16;
     const size_t red = (size_t)BAND_THREADS * 2 * sizeof(double);
-    size_t smem = BandSmem(R, tp, wpair, raw, auxpair).bytes;
+    size_t smem = BandSmem(R, tp, wpair, raw, auxpair, mom).bytes;
     if (smem < red) smem = red;
     if (smem > 200 * 1024) return false;
     int per_sm = 0;

@@ -105,7 +105,9 @@ __global__ void __launch_bounds__(BT_MAX_THREADS, 1) k_leja_tma_batched(const Ba
     using Raw = typename PairT<PREC>::Raw;
     using RecT = Rec<PREC>;
     constexpr int MB = base_mode(MODE);
-    constexpr bool MOM = mom_mode(MODE);   // (see MODE_MOMENT: the aux rows are W_{j-1})
+    constexpr bool MOM = mom_mode(MODE);   // (see MODE_MOMENT: W_j in w[j & 1], the aux rows and E in w[2])
+    // the buffer of W_j
+    auto w_buf = [](int j) { return MOM ? j & 1 : j == 0 ? 0 : ((j & 1) ? 1 : 2); };
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) unsigned long long full[TMA_MAX_STAGES];
     __shared__ __align__(8) unsigned long long empty[TMA_MAX_STAGES];
@@ -174,6 +176,7 @@ __global__ void __launch_bounds__(BT_MAX_THREADS, 1) k_leja_tma_batched(const Ba
         float2 fbd = make_float2(0.f, 0.f), fd0d = fbd, fdnd = fbd;
         const void* fwin = nullptr;
         void* fwout = nullptr;
+        void* feout = nullptr;
         void* faux = nullptr;
         const int32_t* fcol = nullptr;
         const void* fvals = nullptr;
@@ -206,9 +209,10 @@ __global__ void __launch_bounds__(BT_MAX_THREADS, 1) k_leja_tma_batched(const Ba
                     fbd = cfd[2 * d.x];
                     fd0d = cfd[1];
                     fdnd = cfd[2 * (d.x + 1) + 1];
-                    const int buf = d.x == 0 ? 0 : ((d.x & 1) ? 1 : 2);
+                    const int buf = w_buf(d.x);
                     fwin = M->w[buf];
-                    fwout = M->w[(d.x & 1) ? 2 : 1];
+                    fwout = M->w[w_buf(d.x + 1)];
+                    if constexpr (MOM) feout = M->w[2];
                     faux = MB == MODE_ACCUM ? M->p : static_cast<void*>(M->partials);
                     fcol = M->colind;
                     fvals = M->vals;
@@ -217,7 +221,7 @@ __global__ void __launch_bounds__(BT_MAX_THREADS, 1) k_leja_tma_batched(const Ba
                     if (d.x > 0) farr = ld_relaxed_u64(&bp.arrived[d.y]);
                     prefetch_map(&M->win[buf]);
                     prefetch_map(&M->gat[buf]);
-                    if (MB == MODE_DOT || d.x > 0) prefetch_map(&M->aux[MOM && d.x > 1 ? ((d.x & 1) ? 2 : 1) : 0]);
+                    if ((MB == MODE_DOT && !MOM) || d.x > 0) prefetch_map(&M->aux);
                 }
             }
             // runs of consecutive tickets with the same (step, matrix) inside a batch share one
@@ -237,7 +241,8 @@ __global__ void __launch_bounds__(BT_MAX_THREADS, 1) k_leja_tma_batched(const Ba
                 const uint32_t bar = smem_u32(&gbar[slot]);
                 if (fj >= 0) {
                     it.beta = fbeta;
-                    it.d0 = fd0;
+                    if constexpr (MOM) it.eout = feout;
+                    else it.d0 = fd0;
                     it.dn = fdn;
                     it.beta_df = fbd;
                     it.d0_df = fd0d;
@@ -342,7 +347,7 @@ __global__ void __launch_bounds__(BT_MAX_THREADS, 1) k_leja_tma_batched(const Ba
             }
             const BatchTmaMat* M = bp.mats + i;
             const int t = ring[slot].t, gt = ring[slot].gt, ng = ring[slot].ng, nw = ring[slot].nw;
-            const int buf = j == 0 ? 0 : ((j & 1) ? 1 : 2);
+            const int buf = w_buf(j);
             const bool has_aux = (MB == MODE_DOT && !MOM) || j > 0;
             const int ngr = (ng + 3) >> 2;
             unsigned char* st = smem + s * q.stage_bytes;
@@ -355,8 +360,7 @@ __global__ void __launch_bounds__(BT_MAX_THREADS, 1) k_leja_tma_batched(const Ba
                 mbar_arrive_expect_tx(bar, bytes);
                 bulk_copy(smem_u32(st + q.off_desc), bp.desc + (size_t)gt * q.desc_stride, dbytes16, bar);
                 tma_load_rows(smem_u32(st), &M->win[buf], t * R - TMA_HALO, bar);
-                // (moments: W_{j-1} lies in W_0 at the second step, then where this step's W_{j+1} goes)
-                if (has_aux) tma_load_rows(smem_u32(st + q.off_aux), &M->aux[MOM && j > 1 ? ((j & 1) ? 2 : 1) : 0], t * R, bar);
+                if (has_aux) tma_load_rows(smem_u32(st + q.off_aux), &M->aux, t * R, bar);
             }
             const int* gcs = reinterpret_cast<const int*>(gring + slot * q.gcol_stride);
             // extra windows (runs of far columns) in the first gather slots, then the gathers
@@ -549,17 +553,18 @@ __global__ void __launch_bounds__(BT_MAX_THREADS, 1) k_leja_tma_batched(const Ba
             StepParams p{};
             p.first = (j == 0);
             p.beta = sitem[s].beta;
-            p.d0 = sitem[s].d0;
+            if constexpr (!MOM) p.d0 = sitem[s].d0;
             p.dn = sitem[s].dn;
             p.beta_df = sitem[s].beta_df;
             p.d0_df = sitem[s].d0_df;
             p.dn_df = sitem[s].dn_df;
-            p.mcoef = j == 1 ? -2.f : -1.f;
+            p.mcoef = p.first ? -2.f : -1.f;
             const StepScalars<PREC> S(p, cp);
             if (active && r < n) {
                 const WP* __restrict__ win = static_cast<const WP*>(sitem[s].win);
                 WP* wout = static_cast<WP*>(sitem[s].wout);
                 PP* pblk = static_cast<PP*>(sitem[s].aux);
+                WP* eout = MOM ? static_cast<WP*>(sitem[s].eout) : nullptr;
                 const int* srp = reinterpret_cast<const int*>(st + q.off_desc);
                 const RecT* rec = reinterpret_cast<const RecT*>(st + q.off_desc + q.hdr_bytes);
                 const int k0 = srp[rlane], k1 = srp[rlane + 1];
@@ -593,7 +598,8 @@ __global__ void __launch_bounds__(BT_MAX_THREADS, 1) k_leja_tma_batched(const Ba
                         row_mac<PREC>(A, expand(vals[z0 + kk]), x);
                     }
                 }
-                row_epilogue<PREC, MODE>(p, S, A, wr, vr, po, wout + (size_t)r * ldq + cp, pblk + (size_t)r * ldpq + cp, TP);
+                row_epilogue<PREC, MODE>(p, S, A, wr, vr, po, wout + (size_t)r * ldq + cp, pblk + (size_t)r * ldpq + cp, TP, WP{},
+                                         eout + (size_t)r * ldq + cp);
             }
             if constexpr (MB == MODE_DOT) {
                 // At the end of a run, write the run's per-thread trace terms to the next of BT_NRB buffers,

@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(step_max_threads<PREC>(), 2) k_leja_step(const
     const WP* __restrict__ win = static_cast<const WP*>(p.win);
     WP* wout = static_cast<WP*>(p.wout);
     const Raw* __restrict__ vals = static_cast<const Raw*>(p.vals);
-    const WP* vblk = static_cast<const WP*>(p.v);   // (may be wout: moments)
+    const WP* vblk = static_cast<const WP*>(p.v);   // (may be eout: moments)
     PP* __restrict__ pblk = static_cast<PP*>(p.p);
     const int* __restrict__ rowptr = p.rowptr;
     const int* __restrict__ colind = p.colind;
@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(step_max_threads<PREC>(), 2) k_leja_step(const
                 if constexpr (MB == MODE_ACCUM) {
                     if (!p.first) po = pblk[(size_t)r * ldpq + cp];
                 }
-                // (moments: W_{j-1}, whose place this thread's W_{j+1} takes below)
+                // (moments: E_{j-1}, whose place this thread's E_j takes below)
                 if constexpr (mom_mode(MODE)) {
                     if (!p.first) vr = vblk[(size_t)r * ldvq + cp];
                 } else if constexpr (MB == MODE_DOT || MB == MODE_ADJ) {

@@ -84,7 +84,7 @@ struct StepScalars {
     f2x ch2, cl2, nch2, cf2;
     double cadj20, cadj21;   // ADJ: the coefficients of the second block
     f2x c2h2, c2l2, nc2h2;
-    f2x mc2;           // DOT_MOM: the factor of W_{j-1}
+    f2x mc2;           // DOT_MOM: the factor of W_j in W_{j+1}
     double mcd;
     double dn0, dn1;   // d_{j+1} per column (zero in retired columns under the stopping rule)
     double betad, d0d;   // beta_j and d_0 (FP64)
@@ -151,8 +151,8 @@ struct StepScalars {
 
 // Epilogue of one row: W_{j+1} = acc + beta_j W_j[r] (+ coef U[r] in the adjoint), stored to
 // *wout; pass 1: *pout = (first ? d_0 W_j[r] : po) + d_{j+1} W_{j+1}; pass 2: trace terms
-// V[r] . W_{j+1}[r] (and V[r] . W_j[r] on the first step), or in the moment form (vr = W_{j-1}[r])
-// W_j[r] . W_{j+1}[r] and ||W_{j+1}[r]||^2 (and ||W_0[r]||^2); FP32-mixed: vr = E_{j-1}[r], E_j[r] to *eout.
+// V[r] . W_{j+1}[r] (and V[r] . W_j[r] on the first step), or in the moment form (vr = E_{j-1}[r], E_j[r] to
+// *eout) W_j[r] . W_{j+1}[r] and ||W_{j+1}[r]||^2 (and ||W_0[r]||^2).
 template <int PREC, int MODE>
 __device__ __forceinline__ void row_epilogue(const StepParams& p, const StepScalars<PREC>& S, RowAcc& A,
                                              const typename PairT<PREC>::W& wr, const typename PairT<PREC>::W& vr,
@@ -168,9 +168,12 @@ __device__ __forceinline__ void row_epilogue(const StepParams& p, const StepScal
         double w0 = fma(S.betad, wr.x, A.a0), w1 = fma(S.betad, wr.y, A.a1);
         if constexpr (MOM) {
             if (!p.first) {
-                w0 = fma(S.mcd, vr.x, w0);
-                w1 = fma(S.mcd, vr.y, w1);
+                w0 -= vr.x;
+                w1 -= vr.y;
             }
+            *eout = make_double2(w0, w1);
+            w0 = fma(S.mcd, wr.x, w0);
+            w1 = fma(S.mcd, wr.y, w1);
         }
         if constexpr (MB == MODE_ADJ) {
             w0 = fma(S.cadj0, vr.x, w0);
@@ -201,7 +204,10 @@ __device__ __forceinline__ void row_epilogue(const StepParams& p, const StepScal
     } else if constexpr (PREC == LL_PREC_DF64) {
         df2_mac(A.ah, A.al, S.bh2, S.bl2, S.nbh2, wr.x, wr.y);
         if constexpr (MOM) {
-            if (!p.first) df2_add_pow2(A.ah, A.al, S.mc2, vr.x, vr.y);
+            if (!p.first) df2_add_pow2(A.ah, A.al, f2_pack(-1.f, -1.f), vr.x, vr.y);
+            df2_norm(A.ah, A.al, A.ah, A.al);
+            *eout = make_ulonglong2(A.ah, A.al);
+            df2_add_pow2(A.ah, A.al, S.mc2, wr.x, wr.y);
         }
         if constexpr (MB == MODE_ADJ) {
             df2_mac_pp(A.ah, A.al, S.ch2, S.cl2, S.nch2, vr.x, vr.y);
@@ -232,7 +238,6 @@ __device__ __forceinline__ void row_epilogue(const StepParams& p, const StepScal
     } else {  // LL_PREC_F32_MIXED
         f2x wn = f2_fma(S.beta2, wr, A.ah);
         if constexpr (MOM) {
-            // through the sums E_j = D_{j+1} + D_j (see MODE_MOMENT): vr = E_{j-1}
             if (!p.first) wn = f2_sub(wn, vr);
             *eout = wn;
             wn = f2_fma(S.mc2, wr, wn);

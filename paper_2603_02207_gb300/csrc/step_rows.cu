@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, 2) k_leja_rows(const StepParams 
     const WP* __restrict__ win = static_cast<const WP*>(p.win);
     WP* wout = static_cast<WP*>(p.wout);
     const Raw* __restrict__ vals = static_cast<const Raw*>(p.vals);
-    const WP* vblk = static_cast<const WP*>(p.v);   // (may be wout: moments)
+    const WP* vblk = static_cast<const WP*>(p.v);   // (may be eout: moments)
     PP* pblk = static_cast<PP*>(p.p);
     const int* __restrict__ rowptr = p.rowptr;
     const int* __restrict__ colind = p.colind;
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, 2) k_leja_rows(const StepParams 
 #pragma unroll
         for (int z = 0; z < Q; ++z)
             if (has[z]) *reinterpret_cast<X*>(wout + (size_t)r * ldq + cp0 + z * PU) = wn[z];
-        if constexpr (PREC == LL_PREC_F32_MIXED && mom_mode(MODE)) {
+        if constexpr (mom_mode(MODE)) {
 #pragma unroll
             for (int z = 0; z < Q; ++z)
                 if (has[z]) *reinterpret_cast<X*>(static_cast<WP*>(p.eout) + (size_t)r * ldq + cp0 + z * PU) = en[z];

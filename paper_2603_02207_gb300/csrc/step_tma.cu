@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(TMA_MAX_THREADS, 1)
                 for (int qq = 0; qq < NP; ++qq)
                     row_epilogue<PREC, MODE>(p, qq == 0 ? S0 : S1, A[qq], wr[qq], vr[qq], po[qq], &wn[qq], &pn[qq], T[qq], v2r[qq], &en[qq]);
                 st_pairs<NP>(wo, wn);
-                if constexpr (PREC == LL_PREC_F32_MIXED && mom_mode(MODE)) st_pairs<NP>(static_cast<WP*>(p.eout) + (wo - wout), en);
+                if constexpr (mom_mode(MODE)) st_pairs<NP>(static_cast<WP*>(p.eout) + (wo - wout), en);
                 if constexpr (MB == MODE_ACCUM) {
 #pragma unroll
                     for (int qq = 0; qq < NP; ++qq) po_ptr[qq] = pn[qq];

@@ -370,10 +370,10 @@ constexpr int BT_MAX_THREADS = 512 + 96;   // consumers, then the producer, free
 struct BatchTmaMat {
     CUtensorMap gat[3];          // gather maps (one-row box) over W_0 (S or V), wa, wb
     CUtensorMap win[3];          // window maps (R + 2 HALO rows) over the same buffers
-    CUtensorMap aux[3];          // R rows of P (pass 1) or V (pass 2); moments: of W_0, wa, wb
+    CUtensorMap aux;             // R rows of P (pass 1) or V (pass 2); moments: of E
     const int32_t* colind;
     const void* vals;            // prepared values (direct loads past the records)
-    void* w[3];                  // W_0, wa, wb
+    void* w[3];                  // W_0, wa, wb (moments: W_{2j}, W_{2j+1}, E)
     void* p;                     // pass 1: P
     double* partials;            // pass 2: per tile trace partials, slots * T * b (FP64; double-float
                                  // pairs, one float2 per 8 bytes, in the DF64 and FP32 modes)
@@ -386,7 +386,11 @@ struct BatchTmaMat {
 // ring: the step scalars and the matrix's pointers, so that no consumer reads global memory
 // before its rows' operands.
 struct BItem {
-    double beta, d0, dn;         // beta_j, d_0, d_{j+1}
+    double beta, dn;             // beta_j, d_{j+1}
+    union {
+        double d0;               // d_0
+        void* eout;              // moments: E
+    };
     float2 beta_df, d0_df, dn_df;   // the same as double-float pairs
     const void* win;             // W_j (direct loads)
     void* wout;                  // W_{j+1}

@@ -44,3 +44,19 @@ def test_choice_is_not_taken_over_by_another_kind_of_matrix(L, first):
         got = L.ll_apply_poly(h, dA, lo, hi, 4, V, "f32")
         assert h.debug_families_run()[0] == ("rows" if name == "irregular" else "step")
         assert torch.equal(got, L.ll_apply_poly(g, dA, lo, hi, 4, V, "f32")), name
+
+
+def test_stopping_rule_takes_a_timed_kernel_that_has_it(L):
+    """On an irregular matrix the row kernel is the fixed-degree choice but has no stopping rule; the rule's passes take
+    the TMA kernel (eight times as fast there as the register kernel's default shape)."""
+    P = powerlaw_laplacian(1 << 17, seed=1)
+    dA, hi = L.DeviceCSR.from_host(P, "f32"), O.gershgorin(P)[1]
+    h, g = L.Handle(), L.Handle()
+    o = dict(degree=10, probes=60, seed=1, precision="f32", reorder="none")
+    L.ll_logdet_forward(h, dA, 0.01, hi, L.options(**o))
+    assert h.debug_families_run()[0] == "rows"
+    got = L.ll_logdet_forward(h, dA, 0.01, hi, L.options(tol=1e-30, **o))
+    i = h.info()
+    assert (i["kernel_pass1"], i["kernel_pass2"]) == (L.STEP_KERNELS["tma"],) * 2
+    want = L.ll_logdet_forward(g, dA, 0.01, hi, L.options(tol=1e-30, step_kernel="gather", **o))
+    assert abs(got - want) <= 1e-9 * abs(want)

@@ -60,3 +60,29 @@ def test_stopping_rule_takes_a_timed_kernel_that_has_it(L):
     assert (i["kernel_pass1"], i["kernel_pass2"]) == (L.STEP_KERNELS["tma"],) * 2
     want = L.ll_logdet_forward(g, dA, 0.01, hi, L.options(tol=1e-30, step_kernel="gather", **o))
     assert abs(got - want) <= 1e-9 * abs(want)
+
+
+def test_wide_stencil_gets_its_far_windows(L):
+    """An 81-point stencil: rows of more than 64 entries, whose far entries lie on diagonal runs. With windows for
+    the runs a stage holds tens of rows; with a gather for each of 72 far entries a row, four."""
+    N = 200
+    g = np.arange(N * N).reshape(N, N)
+    row, col = [], []
+    for dy in range(-4, 5):
+        for dx in range(-4, 5):
+            a = g[max(0, -dy): N - max(0, dy), max(0, -dx): N - max(0, dx)].ravel()
+            row.append(a)
+            col.append(a + dy * N + dx)
+    row, col = np.concatenate(row), np.concatenate(col)
+    o = np.lexsort((col, row))
+    row, col = row[o], col[o]
+    rowptr = np.concatenate([[0], np.cumsum(np.bincount(row, minlength=N * N))]).astype(np.int32)
+    dA = L.DeviceCSR.from_host(CSR(N * N, rowptr, col.astype(np.int32), np.where(row == col, 100.0, -1.0)), "f32")
+    h, r = L.Handle(), L.Handle()
+    o = dict(degree=10, probes=30, seed=1, precision="f32")
+    got = L.ll_logdet_forward(h, dA, 15.0, 185.0, L.options(step_kernel="tma", **o))
+    i = h.info()
+    assert (i["kernel_pass1"], i["kernel_pass2"]) == (L.STEP_KERNELS["tma"],) * 2
+    assert min(i["rows_pass1"], i["rows_pass2"]) >= 16
+    want = L.ll_logdet_forward(r, dA, 15.0, 185.0, L.options(step_kernel="gather", **o))
+    assert abs(got - want) <= 1e-9 * abs(want)

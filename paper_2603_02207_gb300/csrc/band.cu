@@ -235,9 +235,9 @@ __global__ void k_to_dia(const int32_t* rowptr, const int32_t* colind, const Raw
 
 template <int PREC, int MODE>
 int band_occupancy(size_t smem) {
-    cudaFuncSetAttribute(k_leja_band<PREC, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_leja_band<PREC, MODE>, BAND_THREADS, smem) != cudaSuccess) {
+    if (allow_smem(k_leja_band<PREC, MODE>) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_leja_band<PREC, MODE>, BAND_THREADS, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -246,7 +246,7 @@ int band_occupancy(size_t smem) {
 
 template <int PREC, int MODE>
 cudaError_t band_launch(const BandLaunch& L, const BandParams& p, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(k_leja_band<PREC, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
+    cudaError_t e = allow_smem(k_leja_band<PREC, MODE>);
     if (e != cudaSuccess) return e;
     k_leja_band<PREC, MODE><<<L.grid, BAND_THREADS, L.smem, s>>>(p);
     return cudaGetLastError();

@@ -684,7 +684,7 @@ namespace {
 
 template <int PREC, int MODE>
 cudaError_t launch_bt_typed(const BatchTmaParams& bp, const BatchTmaLaunch& L, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(k_leja_tma_batched<PREC, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
+    cudaError_t e = allow_smem(k_leja_tma_batched<PREC, MODE>);
     if (e != cudaSuccess) return e;
     k_leja_tma_batched<PREC, MODE><<<L.grid, L.threads, L.smem, s>>>(bp, (int)L.off_red, (int)L.off_tab);
     return cudaGetLastError();
@@ -692,7 +692,7 @@ cudaError_t launch_bt_typed(const BatchTmaParams& bp, const BatchTmaLaunch& L, c
 
 template <int PREC, int MODE>
 int occupancy_bt(int threads, size_t smem) {
-    if (cudaFuncSetAttribute(k_leja_tma_batched<PREC, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    if (allow_smem(k_leja_tma_batched<PREC, MODE>) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }

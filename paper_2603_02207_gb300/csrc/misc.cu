@@ -1,6 +1,9 @@
 // Probe generation, CSR validation, Gershgorin bounds, value preparation, block conversions and
 // the FP64 pieces of the power iteration.
 #include <algorithm>
+#include <mutex>
+#include <set>
+#include <utility>
 
 #include "common.cuh"
 #include "gauss.cuh"
@@ -73,6 +76,25 @@ cudaError_t launch_probes(int out_type, int kind, uint64_t seed, int stream_id, 
         default: k_probes<dfp><<<(int)blocks, threads, 0, s>>>(kind, seed, stream_id, n, cols, pad, (dfp*)out, ld, rowmap); break;
     }
     return cudaGetLastError();
+}
+
+// ------------------------------------------------------------------------------- launch limits
+cudaError_t allow_smem(const void* kernel, bool clusters) {
+    static std::mutex lock;
+    static std::set<std::pair<int, const void*>> done;
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> g(lock);
+    if (done.count({dev, kernel})) return cudaSuccess;
+    cudaFuncAttributes at;
+    if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+    if ((e = cudaFuncGetAttributes(&at, kernel)) != cudaSuccess) return e;
+    const int dynamic = optin - (int)at.sharedSizeBytes;
+    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dynamic)) != cudaSuccess) return e;
+    if (clusters && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
+    done.insert({dev, kernel});
+    return cudaSuccess;
 }
 
 // ----------------------------------------------------------------------------- CSR validation

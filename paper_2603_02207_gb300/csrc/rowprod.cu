@@ -250,7 +250,7 @@ cudaError_t rows_df_launch(RowProdParams q, cudaStream_t s) {
     q.TR = 32 * RB;
     const int warps = std::min(std::max(CGT * RB / 2, 1), RP_MAX_WARPS);
     const size_t smem = mats + q.bufs * stage(RB);
-    cudaError_t e = cudaFuncSetAttribute(k_rows_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(smem, 48 * 1024));
+    cudaError_t e = allow_smem(k_rows_df);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rows_df, warps * 32, smem);
@@ -294,7 +294,7 @@ cudaError_t launch_rows_basis(const void* Q1, long long ldx, int n, int k, const
 
 cudaError_t launch_small_project(const double* Rinv, int k, const double* C, int kc, double* Cp, cudaStream_t s) {
     const size_t smem = ((size_t)k * (k + 1) + 8 * k) * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(k_small_project, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(smem, 48 * 1024));
+    cudaError_t e = allow_smem(k_small_project);
     if (e != cudaSuccess) return e;
     k_small_project<<<(kc + 3) / 4, 128, smem, s>>>(Rinv, k, C, kc, Cp);
     return cudaGetLastError();

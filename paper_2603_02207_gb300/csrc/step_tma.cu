@@ -504,9 +504,9 @@ namespace {
 
 template <int PREC, int MODE, int NP>
 int occupancy_tma(int threads, size_t smem) {
-    cudaFuncSetAttribute(k_leja_tma<PREC, MODE, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_leja_tma<PREC, MODE, NP>, threads, smem) != cudaSuccess) {
+    if (allow_smem(k_leja_tma<PREC, MODE, NP>) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_leja_tma<PREC, MODE, NP>, threads, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -516,7 +516,7 @@ int occupancy_tma(int threads, size_t smem) {
 template <int PREC, int MODE, int NP>
 cudaError_t launch_tma_typed(const TmaLaunch& L, const CUtensorMap& g, const CUtensorMap& o, const CUtensorMap& a,
                              const StepParams& p, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(k_leja_tma<PREC, MODE, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
+    cudaError_t e = allow_smem(k_leja_tma<PREC, MODE, NP>);
     if (e != cudaSuccess) return e;
     return launch_step_kernel(k_leja_tma<PREC, MODE, NP>, L.grid, L.threads, L.smem, s, g, o, a, p, L.q);
 }

@@ -62,3 +62,28 @@ def test_auto_forward_matches_oracle_and_step_kernels(L, name, probes, prec):
     assert abs(e[0] - ref) <= (1e-12 if prec != "f32" else 1e-9) * abs(ref)
     want = O.logdet_leja(A, lo, hi, 21, probes, 3, f32=(prec == "f32"))["estimate"]
     assert abs(e[0] - want) <= TOL[prec] * abs(want)
+
+
+@pytest.mark.parametrize("prec", ["f32", "df64"])
+def test_cluster_trace_sums_keep_fp64_accuracy(L, prec):
+    """One warp, one row a lane in both kernels, so that the same 25 terms are added: 8 2^-53 of the sum of their
+    sizes, four times the usual error of two FP64 trees (a sum in double-float is off by up to 2^-48 of it)."""
+    A = laplacian_2d(5, 0.3)
+    dA = L.DeviceCSR.from_host(A, "f32" if prec == "f32" else "f64")
+    lo, hi = 0.3, 8.3
+    c, g = (lo / 0.3 + hi / 0.3) / 2, (hi / 0.3 - lo / 0.3) / 4
+    d, _ = L.ll_divided_differences(lo / 0.3, hi / 0.3, 1)
+    M = O._scipy(A)
+    worst = 0.0
+    for seed in range(60):
+        o = dict(degree=1, probes=1, seed=seed, precision=prec, estimator="hutchinson", keep_for_backward=True, probe_kind="gaussian")
+        h, r = L.Handle(), L.Handle()
+        h.debug_family("cluster")
+        L.ll_logdet_forward(h, dA, lo, hi, L.options(**o))
+        assert h.debug_families_run()[1] == "cluster"
+        L.ll_logdet_forward(r, dA, lo, hi, L.options(step_kernel="gather", rows_per_thread=1, **o))
+        v = L.ll_probes(h, "gaussian", seed, 1, A.n, 1).cpu().numpy()
+        w = M @ v / (0.3 * g) - (c / g + 2.0) * v
+        size = (abs(d[0]) * np.abs(v * v) + abs(d[1]) * np.abs(v * w)).sum()
+        worst = max(worst, abs(h.info()["trace_res"] - r.info()["trace_res"]) / size)
+    assert worst <= 8 * 2.0 ** -53

@@ -68,10 +68,11 @@ __device__ __forceinline__ double df_to_double(float2 v) { return (double)v.x + 
 
 // A double as an unevaluated float pair hi + lo, from its bit fields with integer operations and
 // one integer-to-float conversion (GB300 runs FP64 instructions, conversions from double among
-// them, at a small fraction of the FP32 rate): hi takes the sign, the exponent and the leading 23
-// stored mantissa bits (truncated), lo the remaining 29 bits rounded to 24, scaled by
-// 2^(e - 52). |x - hi - lo| <= 2^-47 |x|. Values outside the float pair's exponent range (zero,
-// subnormals, |x| >= 2^128, inf, nan) take the plain conversion and lo = 0.
+// them, at a small fraction of the FP32 rate): hi is x rounded to 24 bits (ties away from zero), lo the rest,
+// at most half of hi's last place, rounded to 24 bits: |x - hi - lo| <= 2^-49 |x|. (A hi cut off instead leaves lo
+// of one sign and twice the size; products that leave out lo lo then gave squares 2.6e-15 too small on average,
+// 6e-16 so.) Values outside the float pair's exponent range (zero, subnormals, |x| >= 2^128, inf, nan) take the
+// plain conversion and lo = 0.
 __device__ __forceinline__ void split_bits(double x, float& h, float& l) {
     const unsigned long long u = (unsigned long long)__double_as_longlong(x);
     const unsigned int hw = (unsigned int)(u >> 32);
@@ -83,8 +84,10 @@ __device__ __forceinline__ void split_bits(double x, float& h, float& l) {
     }
     const unsigned int sign = hw & 0x80000000u;
     const unsigned long long m = u & 0xFFFFFFFFFFFFFull;
-    h = __uint_as_float(sign | ((unsigned int)(e + 127) << 23) | (unsigned int)(m >> 29));
-    const float lf = __uint2float_rn((unsigned int)(m & 0x1FFFFFFFull));
+    const int rest = (int)(m & 0x1FFFFFFFull);
+    const int up = e < 127 ? rest >> 28 : 0;   // (the carry may reach the exponent; not past the largest float)
+    h = __uint_as_float((sign | ((unsigned int)(e + 127) << 23) | (unsigned int)(m >> 29)) + (unsigned int)up);
+    const float lf = __int2float_rn(rest - (up << 29));
     l = ldexpf(sign ? -lf : lf, e - 52);
 }
 
@@ -137,6 +140,11 @@ __device__ __forceinline__ void df2_mac(f2x& sh, f2x& sl, f2x ah2, f2x al2, f2x 
     const f2x t3 = f2_add(q, bb);
     sl = f2_add(sl, f2_add(f2_sub(t2, t3), e));
     sh = s;
+}
+// The same with the product of the trailing parts (2^-48 of the whole, of one sign in a square)
+__device__ __forceinline__ void df2_mac_ll(f2x& sh, f2x& sl, f2x ah2, f2x al2, f2x nah2, f2x xh2, f2x xl2) {
+    df2_mac(sh, sl, ah2, al2, nah2, xh2, xl2);
+    sl = f2_fma(al2, xl2, sl);
 }
 // (sh, sl) += a * x on both lanes for a double-float scalar a and plain float pairs x (lo = 0).
 __device__ __forceinline__ void df2_mac_f(f2x& sh, f2x& sl, f2x ah2, f2x al2, f2x nah2, f2x x2) {

@@ -212,8 +212,13 @@ __global__ void __launch_bounds__(QR_THREADS) k_gram(long long ldx, int kx, long
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const f2x a2h = f2_pack(ah[i], ah[i]), a2l = f2_pack(al[i], al[i]), na2h = f2_pack(-ah[i], -ah[i]);
-                    df2_mac(h2[2 * i], l2[2 * i], a2h, a2l, na2h, c0h, c0l);
-                    df2_mac(h2[2 * i + 1], l2[2 * i + 1], a2h, a2l, na2h, c1h, c1l);
+                    if constexpr (std::is_same<TX, double>::value) {
+                        df2_mac_ll(h2[2 * i], l2[2 * i], a2h, a2l, na2h, c0h, c0l);
+                        df2_mac_ll(h2[2 * i + 1], l2[2 * i + 1], a2h, a2l, na2h, c1h, c1l);
+                    } else {
+                        df2_mac(h2[2 * i], l2[2 * i], a2h, a2l, na2h, c0h, c0l);
+                        df2_mac(h2[2 * i + 1], l2[2 * i + 1], a2h, a2l, na2h, c1h, c1l);
+                    }
                 }
             }
         }

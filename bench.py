@@ -15,7 +15,7 @@ resident in HBM and larger than L2 (the 553 MB-1.1 GB probe blocks, 175 MB matri
 Usage: python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
        [--precision df64|f64|f32] [--degree M]
 Under torchrun (N > 1) every rank runs an independent replica with seed + rank (weak scaling,
-no data-path collective); rank 0 prints one JSON line.
+no data-path collective); rank 0 prints one JSON line (and the other workloads' figures on stderr).
 """
 from __future__ import annotations
 
@@ -49,19 +49,19 @@ ELEM = {"df64": (8, 8, 8, 8), "f64": (8, 8, 8, 8), "f32": (4, 4, 8, 4)}   # s_A,
 # each kernel on the 96^3 Laplacian (n = 884,736). Traffic grows in proportion to the rows of a stencil
 # matrix, so the full-size value is this figure times n. Only valid for the trace steps of the kernels as
 # captured (profiles/k_leja_tma_moments_96cubed.md).
-TRACE_STEP_DRAM_BYTES_PER_ROW = {("tma", "df64"): (1.052248e9 + 0.432330e9) / 884736,
-                                 ("tma", "f32"): (0.542236e9 + 0.427153e9) / 884736}
+TRACE_STEP_DRAM_BYTES_PER_ROW = {("tma", "df64"): (1.052264e9 + 0.882835e9) / 884736,
+                                 ("tma", "f32"): (0.542241e9 + 0.429853e9) / 884736}
 
 
 def step_bytes(n: int, nnz: int, b: int, prec: str, mode: str) -> int:
     """Algorithmic (compulsory) bytes of one fused Léja step over an n x b block:
     CSR values + column indices + row pointers, W_j read, W_{j+1} written, and
-    P read+written (pass 1: "accum"), V read (pass 2 in m steps: "dot"), or in the moment form ("mom") W_{j-1}
-    read, or FP32-mixed the sums E_j = D_{j+1} + D_j read and written."""
+    P read+written (pass 1: "accum"), V read (pass 2 in m steps: "dot"), or in the moment form ("mom") the
+    sums E_j = D_{j+1} + D_j read and written."""
     s_a, s_w, s_p, s_v = ELEM[prec]
     base = nnz * (s_a + 4) + 4 * (n + 1) + n * b * 2 * s_w
     if mode == "mom":
-        return base + n * b * (2 * s_w if prec == "f32" else s_w)
+        return base + n * b * 2 * s_w
     return base + (n * b * 2 * s_p if mode == "accum" else n * b * s_v)
 
 
@@ -83,6 +83,16 @@ def trace_step_bytes(n: int, nnz: int, b: int, prec: str) -> int:
 def run_bytes(n: int, nnz: int, k: int, m: int, prec: str) -> int:
     """Bytes of the steps that run: m of pass 1 and trace_steps of pass 2."""
     return m * step_bytes(n, nnz, k, prec, "accum") + trace_steps(m, prec, n) * trace_step_bytes(n, nnz, 2 * k, prec)
+
+
+def split_line(line: dict) -> tuple[dict, dict]:
+    """The headline, short enough to be kept whole, and the details beside it (printed on stderr): the workloads
+    and the precisions' phases and rooflines."""
+    keep = ("dtype", "value", "ms_per_step", "hbm_frac_of_measured", "rel_err_vs_exact")
+    short = {key: v for key, v in line.items() if key not in ("workloads", "precisions", "c3_time_to_1e-3")}
+    short["precisions"] = {pr: {key: v[key] for key in keep} for pr, v in line["precisions"].items()}
+    details = {"details": {key: line[key] for key in ("precisions", "workloads", "c3_time_to_1e-3")}}
+    return short, details
 
 
 def load_peaks() -> tuple[dict, str]:
@@ -892,7 +902,9 @@ def main():
         "c3_time_to_1e-3": c3t,
         "gpu_launches": r["launches"], "clocks": r["clocks"], "precisions": precisions, "workloads": extra,
     }
-    print(json.dumps(line))
+    short, details = split_line(line)
+    print(json.dumps(details), file=sys.stderr, flush=True)
+    print(json.dumps(short))
     if world > 1:
         torch.distributed.destroy_process_group()
 

@@ -2,10 +2,11 @@
 column, a group of four and its remainders, the widest block (one tile in shared memory), ragged rows."""
 from __future__ import annotations
 
+import numpy as np
 import pytest
 
 from oracle import logdet as O
-from synth import random_spd
+from synth import diagonal, random_spd
 from tests.gpu_util import lib, rel_err
 
 pytestmark = pytest.mark.gpu
@@ -31,3 +32,19 @@ def test_estimate_and_gradient_match_the_oracle(L, prec, k):
     assert est == pytest.approx(ref["estimate"], rel=2e-5 if prec == "f32" else 1e-9)
     want = O.hutchpp_grad_values(A, lmin, hi, 12, ref["Q"], ref["Gp"])
     assert rel_err(L.ll_logdet_backward(h, dA, 1.0).cpu().numpy(), want) < (1e-4 if prec == "f32" else 1e-9)
+
+
+@pytest.mark.parametrize("prec", ["f64", "df64"])
+def test_ill_conditioned_sketch_keeps_the_deflation(L, prec):
+    """A sketch of condition number 10^6 (the breakdown limit is 10^7): Q^T Q = I and Q^T G' = 0 to 2^-40, a few
+    hundred roundings of 2^-48, and the estimate, whose trace over Q is all of it, to as much of every row."""
+    n, k = 3000, 12
+    logs = np.zeros(n)
+    logs[::n // k] = 10.0 ** np.linspace(0, -4.5, k)
+    h = L.Handle()
+    est = L.ll_logdet_forward(h, L.DeviceCSR.from_host(diagonal(np.exp(logs))), 1.0, float(np.e),
+                              L.options(degree=40, probes=3 * k, seed=4, precision=prec, probe_kind="gaussian", keep_for_backward=True))
+    Q, G = (x.cpu().numpy() for x in L.ll_kept_basis(h))
+    assert np.max(np.abs(Q.T @ Q - np.eye(k))) <= 2.0 ** -40
+    assert np.max(np.abs(Q.T @ G)) <= 2.0 ** -40 * np.sqrt(n)
+    assert abs(est - logs.sum()) <= 2.0 ** -40 * n

@@ -72,12 +72,12 @@ def estimate_bytes(n: int, nnz: int, k: int, m: int, prec: str) -> int:
 
 def trace_steps(m: int, prec: str, n: int) -> int:
     """Steps that a forward's trace pass runs at fixed degree m (no backward kept): ceil(m/2) in the
-    moment form, m for FP32-mixed forwards of fewer than 2^16 rows (or banded)."""
-    return m if prec == "f32" and n < 1 << 16 else (m + 1) // 2
+    moment form, m for FP32-mixed forwards of fewer than 40,000 rows (or banded)."""
+    return m if prec == "f32" and n < 40000 else (m + 1) // 2
 
 
 def trace_step_bytes(n: int, nnz: int, b: int, prec: str) -> int:
-    return step_bytes(n, nnz, b, prec, "dot" if prec == "f32" and n < 1 << 16 else "mom")
+    return step_bytes(n, nnz, b, prec, "dot" if prec == "f32" and n < 40000 else "mom")
 
 
 def run_bytes(n: int, nnz: int, k: int, m: int, prec: str) -> int:

@@ -166,3 +166,42 @@ def test_band_forward_after_a_timed_out_call(L):
                               L.options(degree=8, probes=15, seed=1, precision="df64", qr_gram="tensor"))
     want = O.logdet_leja(A, lo, hi, 8, 15, 1)["estimate"]
     assert abs(got - want) <= TOL["df64"] * abs(want)
+
+
+@pytest.mark.parametrize("prec", ["f64", "df64"])
+@pytest.mark.parametrize("probes", [7, 180, 192])
+def test_band_moments_over_many_launches_and_wide_blocks(L, prec, probes):
+    """More than two launches of the trace pass (E in and out of each), the widest tiles of 32 and of 16 rows; 1e-12 of the
+    one-step kernels, as test_gpu_moments.py's comparisons."""
+    A = _tridiagonal(1500, seed=4)
+    lo, hi = O.gershgorin(A)
+    dA = L.DeviceCSR.from_host(A)
+    est = {}
+    for kernel in ("band", "gather"):
+        h2 = L.Handle()
+        est[kernel] = L.ll_logdet_forward(h2, dA, lo, hi, L.options(degree=41, probes=probes, seed=2, precision=prec, step_kernel=kernel,
+                                                                    estimator="hutchinson"))
+        assert (h2.info()["kernel_pass2"] == L.LL_KERNEL_BAND) == (kernel == "band")
+    assert abs(est["band"] - est["gather"]) <= 1e-12 * (abs(est["gather"]) + A.n)
+
+
+def test_long_band_trace_pass_with_little_memory(L):
+    """The banded pass of more than two launches takes a block of its own; without room for it the step kernels run."""
+    torch = need_gpu()
+    A = pentadiagonal(400_000, seed=5)
+    lo, hi = O.gershgorin(A)
+    dA = L.DeviceCSR.from_host(A)
+    o = dict(probes=90, seed=2, precision="df64", qr_gram="dfloat", use_graph=False)
+    want = L.ll_logdet_forward(L.Handle(), dA, lo, hi, L.options(degree=40, **o))
+    h2 = L.Handle()
+    L.ll_logdet_forward(h2, dA, lo, hi, L.options(degree=16, **o))   # (two launches: every other block is there)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (140 << 20), dtype=torch.uint8, device="cuda")   # a block: 192 MB
+    try:
+        got = L.ll_logdet_forward(h2, dA, lo, hi, L.options(degree=40, **o))
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    assert h2.info()["kernel_pass2"] != L.LL_KERNEL_BAND
+    assert abs(got - want) <= 1e-12 * abs(want)

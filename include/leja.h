@@ -396,6 +396,9 @@ ll_status ll_apply_poly_tol(ll_handle* h, const ll_csr* A, ll_bounds bounds, int
  * With opts->estimator = LL_EST_HUTCHINSON the call skips S, pass 1 and the QR and applies p(A~)
  * to G (probes columns) in the trace pass: estimate = n log sigma + (1/m) tr(G^T p(A~) G).
  * The matrix is device-resident (A). *estimate: host; synchronises `stream`.
+ * A must be symmetric: at fixed degree and with nothing kept, v^T p(A~) v is formed from products of vectors of
+ * half the degree, which holds for a symmetric A only (FP32-mixed: from 40,000 rows, not banded). The call does
+ * not check it; for another matrix the value is not the trace.
  * With opts->keep_for_backward the handle keeps [Q | G'] (Hutchinson: G) for ll_logdet_backward;
  * ll_kept_basis returns LL_ERR_UNSUPPORTED after a Hutchinson forward. */
 ll_status ll_logdet_forward(ll_handle* h, const ll_csr* A, ll_bounds bounds, const ll_options* opts,
@@ -446,8 +449,8 @@ ll_status ll_param_grad(ll_handle* h, const double* grad_values, const double* d
 /* Many independent estimates in one persistent launch per pass (batching, a11): count matrices
  * mats[0..count-1] (device CSR each), bounds b[i], per-matrix degree degrees[i] (NULL = from the
  * bound ratio: m = clamp(ceil(ln 1e6 / ln rho), 10, 250), rho = (sqrt(kappa)+1)/(sqrt(kappa)-1),
- * Proposition 3.1). opts->probes, seed, kind and precision apply to every matrix; matrix i uses
- * seed + i. estimates: host, count doubles; synchronises `stream`.
+ * Proposition 3.1). Every matrix symmetric, as for ll_logdet_forward (F64 and DF64 rest on it). opts->probes,
+ * seed, kind and precision apply to every matrix; matrix i uses seed + i. estimates: host, count doubles; synchronises `stream`.
  * With opts->step_kernel = LL_KERNEL_AUTO the first call for a batch shape (precision, count, k,
  * total rows and entries, largest degree) times the candidate launch shapes on the real operands
  * (the TMA kernel with 512, 384 and 256 consumer threads per pass, i.e. rows per tile, and the
@@ -458,7 +461,7 @@ ll_status ll_logdet_batched(ll_handle* h, const ll_csr* mats, const ll_bounds* b
 
 /* Log-determinants along a matrix pencil (Section 5's GMRF likelihood over a theta grid, where
  * Q(theta) = I + theta Adj): estimates[g] ~ log det A_g for A_g = diag(D) + thetas[g] O, g < t,
- * every A_g symmetric positive definite with spectrum inside bounds[g] (the Léja interval of its
+ * every A_g symmetric (F64 and DF64 rest on it, unchecked) positive definite with spectrum inside bounds[g] (the Léja interval of its
  * own scaling, Section 4) and run at degrees[g] (NULL: opts->degree for every theta). O: device
  * CSR (FP32 or FP64 values; its diagonal entries, if stored, are part of O); D: device, n FP64
  * values; thetas, bounds, degrees, estimates: host arrays of t entries.

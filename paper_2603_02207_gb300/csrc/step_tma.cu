@@ -381,6 +381,14 @@ __global__ void __launch_bounds__(TMA_MAX_THREADS, 1)
 #pragma unroll
                 for (int qq = 0; qq < NP; ++qq)
                     row_epilogue<PREC, MODE>(p, qq == 0 ? S0 : S1, A[qq], wr[qq], vr[qq], po[qq], &wn[qq], &pn[qq], T[qq], v2r[qq], &en[qq]);
+                // (one CTA an SM with few rows a tile: a thread has more than a thousand rows of a large matrix, the
+                // other kernels' threads a tenth of that)
+                if constexpr (PREC == LL_PREC_DF64 && (MB == MODE_DOT || stop_mode(MODE))) {
+                    if (i % 16 == 15) {
+#pragma unroll
+                        for (int qq = 0; qq < NP; ++qq) trace_norm<PREC, MODE>(p, T[qq]);
+                    }
+                }
                 st_pairs<NP>(wo, wn);
                 if constexpr (mom_mode(MODE)) st_pairs<NP>(static_cast<WP*>(p.eout) + (wo - wout), en);
                 if constexpr (MB == MODE_ACCUM) {

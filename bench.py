@@ -49,7 +49,7 @@ ELEM = {"df64": (8, 8, 8, 8), "f64": (8, 8, 8, 8), "f32": (4, 4, 8, 4)}   # s_A,
 # each kernel on the 96^3 Laplacian (n = 884,736). Traffic grows in proportion to the rows of a stencil
 # matrix, so the full-size value is this figure times n. Only valid for the trace steps of the kernels as
 # captured (profiles/k_leja_tma_moments_96cubed.md).
-TRACE_STEP_DRAM_BYTES_PER_ROW = {("tma", "df64"): (1.052264e9 + 0.882835e9) / 884736,
+TRACE_STEP_DRAM_BYTES_PER_ROW = {("tma", "df64"): (1.052430e9 + 0.883082e9) / 884736,
                                  ("tma", "f32"): (0.542241e9 + 0.429853e9) / 884736}
 
 
